@@ -1907,8 +1907,8 @@ static size_t footprint(const gsis_solver *s) {
   if (s->factored)  // one-dimensional Maxwellian factors
     b += nc * (s->vaxis.size() / 2) * factor_table_len(s->nvdf) * 8 + (size_t)s->nslots * 4 + s->vaxis.size() * 8;
   if (!s->general) b += nc * T;
-  if (Sb == 8 && !s->point_set)  // FP64 origin moments: the extra chunk, the table
-    b += (size_t)nc * moment_len(s->nvdf) * 8 + (size_t)s->nslots * 16 * 8 + s->vaxis.size() * 8;
+  if (Sb == 8 && s->nvdf == 1 && !s->point_set)  // FP64 origin moments: the extra chunk, the table
+    b += (size_t)nc * moment_len(1) * 8 + (size_t)s->nslots * 16 * 8 + s->vaxis.size() * 8;
   b += nc * NST * (T + 8);                    // states
   b += nc * (13 + 18 + 18 + 12 + 6 + 6 + 1) * 8;
   b += nc * (6 + 6 + 18 + 15 + 4 + 6 + 2 + 1 + 18 + 6 + 3 + 18 + 72) * 8 + nc * 4;  // synthetic-solve work
@@ -1967,7 +1967,7 @@ static int allocate_and_upload(gsis_solver *s) {
     s->mom_bpc = std::max(1, std::min(64, (s->nblocks + want - 1) / want));
     s->mom_nchunks = (s->nblocks + s->mom_bpc - 1) / s->mom_bpc;
   }
-  s->origin_mom = std::is_same<T, double>::value && !s->point_set;
+  s->origin_mom = std::is_same<T, double>::value && s->nvdf == 1 && !s->point_set;
   A(s->d_mp, (size_t)(s->mom_nchunks + (s->origin_mom ? 1 : 0)) * nc * moment_len(s->nvdf) * sizeof(double));
   const bool tiled = s->kg.tile[0] > 0;
   const int tile_nodes = s->kg.tile[0] + s->kg.tile[1] + s->kg.tile[2];

@@ -196,7 +196,7 @@ cudaError_t launch_wall_prepass(const KinArgs<T, S> &a, const int *wall_cell, co
                                 const double *Z0, double *rho_w, int nslots, cudaStream_t s);
 template <typename T, typename S>
 cudaError_t launch_moments(const KinArgs<T, S> &a, int blocks_per_chunk, int nchunks, double *mp, cudaStream_t s);
-// FP64 storage on a tensor-product grid: moments about the origin into chunks 0..nchunks-1 of mp,
+// FP64 storage on a tensor-product grid, Shakhov: moments about the origin into chunks 0..nchunks-1 of mp,
 // from the table mtab (tiled grids: [block][node of the tile, x then y then z][4] powers of the
 // axis times its weight; else [slot][16]), and the closed-form sums of w phi g^n (from the 1-D
 // grids in vaxis: nodes of x, y, z, then their weights) into chunk nchunks (zeros unless emit)

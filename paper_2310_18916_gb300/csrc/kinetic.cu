@@ -876,32 +876,33 @@ struct __align__(16) double4_16 {
   double x, y, z, w;
 };
 
-// FP64 storage on a tensor-product grid: the moments of the stored f^{n+1/2} about the origin, no
-// exponential: 13 of f0, w (1, xi(3), xi_a xi_b (6), |xi|^2 xi(3)), and for Rykov 4 of f1, w (1, xi(3)).
-// The collision sums sum_v w phi (g^n - f) are assembled per cell by the reduction from the closed
-// form of sum_v w phi g^n (ref_sums_kernel) and these moments.  Row layout as in moments_kernel.
+// FP64 storage on a tensor-product grid, Shakhov: the 13 moments of the stored f^{n+1/2} about the origin,
+// w (1, xi(3), xi_a xi_b (6), |xi|^2 xi(3)), no exponential.  The collision sums sum_v w phi (g^n - f) are
+// assembled per cell by the reduction from the closed form of sum_v w phi g^n (ref_sums_kernel) and
+// these moments.  Row layout as in moments_kernel.  Both cancel where |u| is many thermal speeds (the
+// heat flux loses a factor of |u|^3), so the two VDFs of Rykov, the gas of the hypersonic cases, keep
+// moments_kernel: about the state velocity, with g - f formed point by point (cavity 48^2 with 20^3
+// velocities, moments and reductions 3.8 ms; this form took 0.8).
 
 // Untiled grids: from the per-slot table of the 13 factors (16 doubles per slot, the last three 0),
 // one FMA per moment and point.  Per-block plain sums, compensated (Kahan) across the chunk's blocks.
-template <int NV>
 __global__ void __launch_bounds__(128) moments_origin_kernel(const KinArgs<double, double> A, const double *mtab,
                                                              int blocks_per_chunk, double *mp) {
-  constexpr int N1 = NV == 2 ? NMOM1 : 0, NP = moment_len(NV);
+  constexpr int NP = moment_len(1);
   const int chunk = blockIdx.y;
   const int b0 = chunk * blocks_per_chunk;
   const int nb = min(blocks_per_chunk, A.nblocks - b0);
   const int cell = blockIdx.x * blockDim.x + threadIdx.x;
   if (cell >= A.g.nc) return;
-  MomAcc<double, NMOM + N1> acc;
+  MomAcc<double, NMOM> acc;
   acc.zero();
   for (int bb = 0; bb < nb; ++bb) {
-    double f[VB], f1[NV == 2 ? VB : 1];
+    double f[VB];
     load_block_f<double, double>(A.f + ((size_t)(b0 + bb) * A.g.nc + cell) * VB, f);
-    if constexpr (NV == 2) load_block_f<double, double>(A.f1 + ((size_t)(b0 + bb) * A.g.nc + cell) * VB, f1);
     const double2 *tb = reinterpret_cast<const double2 *>(mtab + (size_t)(b0 + bb) * VB * 16);
-    double sum[NMOM + N1];
+    double sum[NMOM];
 #pragma unroll
-    for (int k = 0; k < NMOM + N1; ++k) sum[k] = 0.0;
+    for (int k = 0; k < NMOM; ++k) sum[k] = 0.0;
 #pragma unroll
     for (int l = 0; l < VB; ++l) {
       double t[14];
@@ -913,8 +914,6 @@ __global__ void __launch_bounds__(128) moments_origin_kernel(const KinArgs<doubl
       }
 #pragma unroll
       for (int k = 0; k < NMOM; ++k) sum[k] = fma(f[l], t[k], sum[k]);
-#pragma unroll
-      for (int k = 0; k < N1; ++k) sum[NMOM + k] = fma(f1[l], t[k], sum[NMOM + k]);
     }
     acc.add(sum);
   }
@@ -923,8 +922,6 @@ __global__ void __launch_bounds__(128) moments_origin_kernel(const KinArgs<doubl
   for (int k = 0; k < NP; ++k) out[k] = 0.0;
 #pragma unroll
   for (int k = 0; k < NMOM; ++k) out[k] = acc.s[k] - acc.c[k];
-#pragma unroll
-  for (int k = 0; k < N1; ++k) out[NMOM + NFF + 1 + k] = acc.s[NMOM + k] - acc.c[NMOM + k];
 }
 
 // Tiled grids: a block of 32 velocities is a TX x TY x TZ tile, so its sums factorise: over x with
@@ -933,20 +930,20 @@ __global__ void __launch_bounds__(128) moments_origin_kernel(const KinArgs<doubl
 // rest on 8 and 2 values).  Plain sums over four tiles (at most 14 additions deep), compensated
 // across them.  The FP64 pipe bounds it: 128^2 cells with 32^3 velocities 13.6 -> 7.8 ms with the
 // reductions.
-template <int TX, int TY, int TZ, int NV>
+template <int TX, int TY, int TZ>
 __global__ void __launch_bounds__(128) moments_tile_kernel(const KinArgs<double, double> A, const double *btab,
                                                            int blocks_per_chunk, double *mp) {
-  constexpr int N1 = NV == 2 ? NMOM1 : 0, NP = moment_len(NV), NN = TX + TY + TZ;
+  constexpr int NP = moment_len(1), NN = TX + TY + TZ;
   const int chunk = blockIdx.y;
   const int b0 = chunk * blocks_per_chunk;
   const int nb = min(blocks_per_chunk, A.nblocks - b0);
   const int cell = blockIdx.x * blockDim.x + threadIdx.x;
   if (cell >= A.g.nc) return;
-  MomAcc<double, NMOM + N1> acc;
+  MomAcc<double, NMOM> acc;
   acc.zero();
-  double S[NMOM + N1];
+  double S[NMOM];
 #pragma unroll
-  for (int k = 0; k < NMOM + N1; ++k) S[k] = 0.0;
+  for (int k = 0; k < NMOM; ++k) S[k] = 0.0;
   for (int bb = 0; bb < nb; ++bb) {
     const size_t at = ((size_t)(b0 + bb) * A.g.nc + cell) * VB;
     const double4_16 *tab = reinterpret_cast<const double4_16 *>(btab + (size_t)(b0 + bb) * NN * 4);
@@ -956,18 +953,17 @@ __global__ void __launch_bounds__(128) moments_tile_kernel(const KinArgs<double,
 #pragma unroll
     for (int iz = 0; iz < TZ; ++iz) {
       // sums over x and y of f times x^p y^q, p + q <= 3
-      double B[4][4], C[2][2];
+      double B[4][4];
 #pragma unroll
       for (int p = 0; p < 4; ++p)
 #pragma unroll
         for (int q = 0; q < 4; ++q) B[p][q] = 0.0;
-      C[0][0] = C[0][1] = C[1][0] = 0.0;
 #pragma unroll
       for (int iy = 0; iy < TY; ++iy) {
         const int l = TX * (iy + TY * iz);
         const double4_16 ty = tab[TX + iy];
         const double py[4] = {ty.x, ty.y, ty.z, ty.w};
-        double a[4] = {0.0, 0.0, 0.0, 0.0}, a1[2] = {0.0, 0.0};
+        double a[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
         for (int ix = 0; ix < TX; ix += 2) {
           const double2 v = __ldcs(reinterpret_cast<const double2 *>(A.f + at + l + ix));
@@ -975,21 +971,11 @@ __global__ void __launch_bounds__(128) moments_tile_kernel(const KinArgs<double,
           a[1] = fma(v.y, tx[ix + 1].y, fma(v.x, tx[ix].y, a[1]));
           a[2] = fma(v.y, tx[ix + 1].z, fma(v.x, tx[ix].z, a[2]));
           a[3] = fma(v.y, tx[ix + 1].w, fma(v.x, tx[ix].w, a[3]));
-          if constexpr (NV == 2) {
-            const double2 u = __ldcs(reinterpret_cast<const double2 *>(A.f1 + at + l + ix));
-            a1[0] = fma(u.y, tx[ix + 1].x, fma(u.x, tx[ix].x, a1[0]));
-            a1[1] = fma(u.y, tx[ix + 1].y, fma(u.x, tx[ix].y, a1[1]));
-          }
         }
 #pragma unroll
         for (int p = 0; p < 4; ++p)
 #pragma unroll
           for (int q = 0; p + q < 4; ++q) B[p][q] = fma(a[p], py[q], B[p][q]);
-        if constexpr (NV == 2) {
-          C[0][0] = fma(a1[0], py[0], C[0][0]);
-          C[0][1] = fma(a1[0], py[1], C[0][1]);
-          C[1][0] = fma(a1[1], py[0], C[1][0]);
-        }
       }
       const double4_16 z = tab[TX + TY + iz];
       S[0] = fma(B[0][0], z.x, S[0]);
@@ -1005,17 +991,11 @@ __global__ void __launch_bounds__(128) moments_tile_kernel(const KinArgs<double,
       S[10] = fma(B[1][0], z.z, fma(B[3][0] + B[1][2], z.x, S[10]));
       S[11] = fma(B[0][1], z.z, fma(B[2][1] + B[0][3], z.x, S[11]));
       S[12] = fma(B[0][0], z.w, fma(B[2][0] + B[0][2], z.y, S[12]));
-      if constexpr (NV == 2) {
-        S[NMOM] = fma(C[0][0], z.x, S[NMOM]);
-        S[NMOM + 1] = fma(C[1][0], z.x, S[NMOM + 1]);
-        S[NMOM + 2] = fma(C[0][1], z.x, S[NMOM + 2]);
-        S[NMOM + 3] = fma(C[0][0], z.y, S[NMOM + 3]);
-      }
     }
     if ((bb & 3) == 3 || bb == nb - 1) {
       acc.add(S);
 #pragma unroll
-      for (int k = 0; k < NMOM + N1; ++k) S[k] = 0.0;
+      for (int k = 0; k < NMOM; ++k) S[k] = 0.0;
     }
   }
   double *out = mp + ((size_t)chunk * A.g.nc + cell) * NP;
@@ -1023,30 +1003,26 @@ __global__ void __launch_bounds__(128) moments_tile_kernel(const KinArgs<double,
   for (int k = 0; k < NP; ++k) out[k] = 0.0;
 #pragma unroll
   for (int k = 0; k < NMOM; ++k) out[k] = acc.s[k] - acc.c[k];
-#pragma unroll
-  for (int k = 0; k < N1; ++k) out[NMOM + NFF + 1 + k] = acc.s[NMOM + k] - acc.c[NMOM + k];
 }
 
-// Closed form of sum_v w phi(xi) g^n(xi), phi = 1, xi(3), |xi|^2/2 (for Rykov of g0, and the sum of
-// g1), on a tensor-product velocity grid: with c = xi - u a Shakhov-type distribution
-// C e^{-|c|^2/T} [1 + a.c (|c|^2/T - 5/2)] is a polynomial in c times a product of one-dimensional
-// Gaussians, so the sum over the grid factorises into the one-dimensional sums m_a[k] = sum_i
-// w_a(i) e^{-c_a(i)^2/T} c_a(i)^k (k <= 5; C in the x ones).  Per cell 3 lanes (Rykov 6: the
-// translational and the equilibrium Maxwellian) take one axis each, then one writes the cell's
-// row of the extra moment chunk (moments 0, collision sums after them); emit = 0 (the velocity
-// shards other than the first) writes zeros, so the sum over shards counts it once.
-template <int NV>
-__global__ void __launch_bounds__(96 * NV) ref_sums_kernel(int nc, const double *st64, const double *vaxis, int nx, int ny,
+// Closed form of sum_v w phi(xi) g^n(xi), phi = 1, xi(3), |xi|^2/2, on a tensor-product velocity grid:
+// with c = xi - u the Shakhov distribution C e^{-|c|^2/T} [1 + a.c (|c|^2/T - 5/2)] is a polynomial in c
+// times a product of one-dimensional Gaussians, so the sum over the grid factorises into the
+// one-dimensional sums m_a[k] = sum_i w_a(i) e^{-c_a(i)^2/T} c_a(i)^k (k <= 5; C in the x ones).  Per
+// cell 3 lanes take one axis each, then one writes the cell's row of the extra moment chunk (moments
+// 0, collision sums after them); emit = 0 (the velocity shards other than the first) writes zeros, so
+// the sum over shards counts it once.
+__global__ void __launch_bounds__(96) ref_sums_kernel(int nc, const double *st64, const double *vaxis, int nx, int ny,
                                                            int nz, int emit, double *row) {
-  constexpr int NP = moment_len(NV);
-  __shared__ double m[NV][3][6][33];
-  const int slot = threadIdx.x & 31, job = threadIdx.x >> 5, set = job / 3, a = job - 3 * set;
+  constexpr int NP = moment_len(1);
+  __shared__ double m[3][6][33];
+  const int slot = threadIdx.x & 31, a = threadIdx.x >> 5;
   const int cell = blockIdx.x * 32 + slot;
   const double *st = st64 + (size_t)cell * NST;
   if (cell < nc && emit) {
     const int n = a == 0 ? nx : (a == 1 ? ny : nz);
     const double *x = vaxis + (a == 0 ? 0 : (a == 1 ? nx : nx + ny)), *w = x + nx + ny + nz;
-    const double u = st[a], invT = st[set ? 24 : 3];
+    const double u = st[a], invT = st[3];
     double s[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     for (int i = 0; i < n; ++i) {
       const double c = x[i] - u;
@@ -1057,69 +1033,53 @@ __global__ void __launch_bounds__(96 * NV) ref_sums_kernel(int nc, const double 
         p *= c;
       }
     }
-    const double C = a == 0 ? st[set ? 25 : 4] : 1.0;
+    const double C = a == 0 ? st[4] : 1.0;
 #pragma unroll
-    for (int k = 0; k < 6; ++k) m[set][a][k][slot] = C * s[k];
+    for (int k = 0; k < 6; ++k) m[a][k][slot] = C * s[k];
   }
   __syncthreads();
-  if (job != 0 || cell >= nc) return;
+  if (a != 0 || cell >= nc) return;
   double *o = row + (size_t)cell * NP;
 #pragma unroll
   for (int k = 0; k < NP; ++k) o[k] = 0.0;
   if (!emit) return;
   const double u[3] = {st[0], st[1], st[2]};
-#pragma unroll
-  for (int q = 0; q < NV; ++q) {
-    auto mono = [&](int px, int py, int pz) { return m[q][0][px][slot] * m[q][1][py][slot] * m[q][2][pz][slot]; };
-    const double invT = st[q ? 24 : 3], *aq = st + (q ? 26 : 12);
-    // sum_v w g c^e for the exponent triple e
-    auto G = [&](int px, int py, int pz) {
-      double t1 = 0.0;
-      for (int b = 0; b < 3; ++b) {
-        const int e[3] = {px + (b == 0), py + (b == 1), pz + (b == 2)};
-        const double s3 = mono(e[0] + 2, e[1], e[2]) + mono(e[0], e[1] + 2, e[2]) + mono(e[0], e[1], e[2] + 2);
-        t1 += aq[b] * (invT * s3 - 2.5 * mono(e[0], e[1], e[2]));
-      }
-      return mono(px, py, pz) + t1;
-    };
-    const double f = NV == 2 ? st[37 + q] : 1.0;  // 1 - 1/Z_r, 1/Z_r
-    const double g1 = f * G(0, 0, 0);
-    const double gc[3] = {f * G(1, 0, 0), f * G(0, 1, 0), f * G(0, 0, 1)};
-    const double gc2 = f * (G(2, 0, 0) + G(0, 2, 0) + G(0, 0, 2));
-    o[NMOM] += g1;
-    for (int b = 0; b < 3; ++b) o[NMOM + 1 + b] += gc[b] + u[b] * g1;
-    double e = 0.5 * gc2 + (u[0] * gc[0] + u[1] * gc[1] + u[2] * gc[2]) +
-               0.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * g1;
-    if constexpr (NV == 2) {
-      // g1: the internal-energy factor times the Shakhov-type part, and its heat-flux term
-      const double *h = st + (q ? 34 : 31), C = st[q ? 25 : 4];
-      const double s1 = st[29 + q] * g1 + f * (h[0] * mono(1, 0, 0) + h[1] * mono(0, 1, 0) + h[2] * mono(0, 0, 1)) / C;
-      o[NMOM + NFF] += s1;
-      e += s1;
+  auto mono = [&](int px, int py, int pz) { return m[0][px][slot] * m[1][py][slot] * m[2][pz][slot]; };
+  const double invT = st[3], *aq = st + 12;
+  // sum_v w g c^e for the exponent triple e
+  auto G = [&](int px, int py, int pz) {
+    double t1 = 0.0;
+    for (int b = 0; b < 3; ++b) {
+      const int e[3] = {px + (b == 0), py + (b == 1), pz + (b == 2)};
+      const double s3 = mono(e[0] + 2, e[1], e[2]) + mono(e[0], e[1] + 2, e[2]) + mono(e[0], e[1], e[2] + 2);
+      t1 += aq[b] * (invT * s3 - 2.5 * mono(e[0], e[1], e[2]));
     }
-    o[NMOM + 4] += e;
-  }
+    return mono(px, py, pz) + t1;
+  };
+  const double g1 = G(0, 0, 0);
+  const double gc[3] = {G(1, 0, 0), G(0, 1, 0), G(0, 0, 1)};
+  const double gc2 = G(2, 0, 0) + G(0, 2, 0) + G(0, 0, 2);
+  o[NMOM] = g1;
+  for (int b = 0; b < 3; ++b) o[NMOM + 1 + b] = gc[b] + u[b] * g1;
+  o[NMOM + 4] = 0.5 * gc2 + (u[0] * gc[0] + u[1] * gc[1] + u[2] * gc[2]) +
+                0.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * g1;
 }
 
 cudaError_t launch_moments_origin(const KinArgs<double, double> &a, const double *mtab, int blocks_per_chunk,
                                   int nchunks, const double *st64, const double *vaxis, const int *nv_axis, int emit,
                                   double *mp, cudaStream_t s) {
   dim3 grid((a.g.nc + 127) / 128, nchunks);
-  auto launch = [&](auto nv) {
-    constexpr int NV = decltype(nv)::value;
-    void (*k)(const KinArgs<double, double>, const double *, int, double *) =
-        a.g.tile[0] == 0   ? moments_origin_kernel<NV>
-        : a.g.tile[0] == 2 ? moments_tile_kernel<2, 4, 4, NV>
-        : a.g.tile[1] == 2 ? moments_tile_kernel<4, 2, 4, NV>
-                           : moments_tile_kernel<4, 4, 2, NV>;
-    k<<<grid, 128, 0, s>>>(a, mtab, blocks_per_chunk, mp);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    ref_sums_kernel<NV><<<(a.g.nc + 31) / 32, 96 * NV, 0, s>>>(a.g.nc, st64, vaxis, nv_axis[0], nv_axis[1], nv_axis[2],
-                                                               emit, mp + (size_t)nchunks * a.g.nc * moment_len(NV));
-    return cudaGetLastError();
-  };
-  return a.nvdf == 2 ? launch(std::integral_constant<int, 2>{}) : launch(std::integral_constant<int, 1>{});
+  void (*k)(const KinArgs<double, double>, const double *, int, double *) =
+      a.g.tile[0] == 0   ? moments_origin_kernel
+      : a.g.tile[0] == 2 ? moments_tile_kernel<2, 4, 4>
+      : a.g.tile[1] == 2 ? moments_tile_kernel<4, 2, 4>
+                         : moments_tile_kernel<4, 4, 2>;
+  k<<<grid, 128, 0, s>>>(a, mtab, blocks_per_chunk, mp);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  ref_sums_kernel<<<(a.g.nc + 31) / 32, 96, 0, s>>>(a.g.nc, st64, vaxis, nv_axis[0], nv_axis[1], nv_axis[2], emit,
+                                                    mp + (size_t)nchunks * a.g.nc * moment_len(1));
+  return cudaGetLastError();
 }
 
 // f_raw = Maxwellian(W0) of each cell at each slot velocity, in the storage precision (the

@@ -40,21 +40,20 @@ __global__ void reduce_moments_kernel(const double *mp, int nchunks, int nc, int
   }
 }
 
-// FP64 storage on a tensor-product grid: chunks 0..nchunks-1 hold sum w f (1, xi, xi xi, |xi|^2 xi)
-// about the origin (Rykov: and sum w f1 (1, xi)), the last chunk sum w phi g^n (and sum w g1).  Per
-// cell: K = V/tau (G - F) with F = sum w phi f (phi = 1, xi, |xi|^2/2; the energy with f1), and the
-// moments about the state velocity u by the binomial shift
+// FP64 storage on a tensor-product grid, Shakhov: chunks 0..nchunks-1 hold sum w f (1, xi, xi xi, |xi|^2 xi)
+// about the origin, the last chunk sum w phi g^n.  Per cell: K = V/tau (G - F) with F = sum w phi f
+// (phi = 1, xi, |xi|^2/2), and the moments about the state velocity u by the binomial shift
 //   M1 = S1 - u S0,  M2_ab = S2_ab - u_a S1_b - u_b S1_a + u_a u_b S0,
 //   M3_a = S3_a - u_a tr S2 - 2 (S2 u)_a + 2 u_a (u.S1) + |u|^2 S1_a - |u|^2 u_a S0.
 // W lanes sum a cell's rows (lane l the rows l, l + W, ..., then a fixed butterfly): 1 where there are
 // few rows, 32 on small meshes, whose many rows are otherwise one long chain (100 cells, 433 rows:
 // 240 us).
-template <int NV, int W>
+template <int W>
 __global__ void __launch_bounds__(128) reduce_origin_kernel(const double *mp, int nrows, int nc, const double *vol,
                                                             const double *st64, double *mom, double *K) {
   const int cell = (blockIdx.x * 128 + threadIdx.x) / W, part = threadIdx.x % W;
   if (cell >= nc) return;  // (a cell's lanes leave together)
-  constexpr int NP = moment_len(NV);
+  constexpr int NP = moment_len(1);
   double S[NP];
 #pragma unroll
   for (int k = 0; k < NP; ++k) S[k] = 0.0;
@@ -76,12 +75,11 @@ __global__ void __launch_bounds__(128) reduce_origin_kernel(const double *mp, in
   const double S0 = S[0], S1[3] = {S[1], S[2], S[3]};
   const double S2[3][3] = {{S[4], S[7], S[8]}, {S[7], S[5], S[9]}, {S[8], S[9], S[6]}};
   const double trS2 = S[4] + S[5] + S[6];
-  const double F1 = NV == 2 ? S[NP - NMOM1] : 0.0;
   double *k6 = K + (size_t)cell * 6;
   k6[0] = kf * (S[NMOM] - S0);
   for (int a = 0; a < 3; ++a) k6[1 + a] = kf * (S[NMOM + 1 + a] - S1[a]);
-  k6[4] = kf * (S[NMOM + 4] - (0.5 * trS2 + F1));
-  k6[5] = NV == 2 ? kf * (S[NP - NMOM1 - 1] - F1) : 0.0;
+  k6[4] = kf * (S[NMOM + 4] - 0.5 * trS2);
+  k6[5] = 0.0;
   const double uS1 = u[0] * S1[0] + u[1] * S1[1] + u[2] * S1[2];
   const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
   double M2[3][3];
@@ -99,9 +97,7 @@ __global__ void __launch_bounds__(128) reduce_origin_kernel(const double *mp, in
   for (int a = 0; a < 3; ++a) {
     const double S2u = S2[a][0] * u[0] + S2[a][1] * u[1] + S2[a][2] * u[2];
     M[10 + a] = S[10 + a] - u[a] * trS2 - 2.0 * S2u + 2.0 * u[a] * uS1 + uu * S1[a] - uu * u[a] * S0;
-    if (NV == 2) M[NMOM + 1 + a] = S[NP - NMOM1 + 1 + a] - u[a] * F1;
   }
-  if (NV == 2) M[NMOM] = F1;
 }
 
 // Outward kinetic wall flux per unit area: the half moving towards the wall from the wall cells'
@@ -147,9 +143,7 @@ cudaError_t launch_reduce(const double *mp, int nchunks, int nvdf, const T *wpar
   if (grid > 152 * 16) grid = 152 * 16;
   if (origin) {
     const bool wide = nchunks > 64;
-    void (*k)(const double *, int, int, const double *, const double *, double *, double *) =
-        nvdf == 2 ? (wide ? reduce_origin_kernel<2, 32> : reduce_origin_kernel<2, 1>)
-                  : (wide ? reduce_origin_kernel<1, 32> : reduce_origin_kernel<1, 1>);
+    const auto k = wide ? reduce_origin_kernel<32> : reduce_origin_kernel<1>;
     const size_t threads = (size_t)g.nc * (wide ? 32 : 1);
     k<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(mp, nchunks + 1, g.nc, vol, st64, mom, K);
   }
