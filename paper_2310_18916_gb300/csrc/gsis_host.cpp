@@ -2126,7 +2126,7 @@ static int allocate_and_upload(gsis_solver *s) {
   }
   if (!rc && !vnode.empty()) rc = s->upload(s->d_vnode, vnode.data(), vnode.size() * sizeof(int));
   std::vector<T> eps2(s->general ? 0 : nc);
-  for (size_t c = 0; c < eps2.size(); ++c) eps2[c] = (T)(s->kg.K3 * s->vol[c]);
+  for (size_t c = 0; c < eps2.size(); ++c) eps2[c] = (T)std::max(s->kg.K3 * s->vol[c], sizeof(T) == 8 ? 1e-250 : 0.0);
   if (!rc && !eps2.empty()) rc = s->upload(s->d_eps2, eps2.data(), nc * sizeof(T));
   if (!rc) rc = s->cuda(cudaStreamSynchronize(s->stream), "sync");  // vnode and eps2 leave scope
   if (!rc) rc = s->upload(s->d_vel64, s->vel64_all.data(), s->vel64_all.size() * sizeof(double));

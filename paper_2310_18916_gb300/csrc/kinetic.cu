@@ -101,7 +101,7 @@ struct KinSmem {
   }
 };
 
-// FX: factored Maxwellians (FP64 on a tensor-product velocity grid).  An FP64 exponential costs 18
+// FX: factored Maxwellians (FP64 on a tensor-product velocity grid).  An FP64 exponential is many
 // instructions of a pipe that retires one warp instruction in 19 cycles per SM, but on a product
 // grid exp(-|xi - u|^2 / T) is the product of three one-dimensional factors, and the polynomials in
 // c = xi - u of the reference distributions are sums of three.  factor_table_kernel writes per cell
@@ -387,7 +387,7 @@ __global__ void kinetic_kernel(const KinArgs<T, S> A) {
       }
       // the implicit diagonal D = 1/dt + 1/tau + the outflow coefficients, then the limiter.  In
       // FP64 one reciprocal r = 1 / (bd D) gives both phi = bn / bd = bn D r and the update's
-      // 1 / D = bd r (an FP64 division costs several FP64 instructions on this GPU)
+      // 1 / D = bd r (bd >= eps^2, which the host keeps far above the smallest normal number)
       T D = st[15];
 #pragma unroll
       for (int a = 0; a < NACT; ++a) D += axi[a] * invh[a];

@@ -8,6 +8,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "fp64_device.cuh"
 #include "gsis_internal.h"
 
 namespace gsis {
@@ -197,15 +198,6 @@ __device__ __forceinline__ T venkat_phi(const Largest<T> &dp, const Largest<T> &
   T bn, bd;
   venkat_parts<T>(dp, dn, d2, eps2, bn, bd);
   return ddiv(bn, bd);
-}
-
-// 1 / x for a normal positive x by two Newton-Raphson steps y += y (1 - x y) from the hardware's
-// approximation of its leading bits: four FP64 instructions instead of seven
-__device__ __forceinline__ double rcp_newton(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
 }
 
 // Per-cell state and colour-entry addresses from 32-bit offsets: a 64-bit multiply by a

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "fp64_device.cuh"
 #include "gsis_internal.h"
 
 namespace gsis {
@@ -72,7 +73,6 @@ __device__ __forceinline__ void grid_sync_part(unsigned *bar, unsigned &epoch, i
 // Comparisons on the integer pipe (an FP64 comparison, min or max costs as much as an FMA on this
 // GPU).  Where the operands are known to be non-negative, the order of their bit patterns as
 // integers is their numeric order (no NaN reaches them on a physical state).
-__device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
 // x > 0 exactly as the FP64 comparison: +0 < bits <= +inf (negative values, -0 and NaN fail)
 __device__ __forceinline__ bool gt0(double x) {
   return (unsigned long long)(dbits(x) - 1) < 0x7ff0000000000000ULL;
@@ -81,67 +81,7 @@ __device__ __forceinline__ bool gt0(double x) {
 __device__ __forceinline__ bool lt_nn(double x, double y) { return dbits(x) < dbits(y); }
 __device__ __forceinline__ double max_nn(double x, double y) { return dbits(x) < dbits(y) ? y : x; }
 
-// 1 / x of a density (normal, positive) by two Newton-Raphson steps y += y (1 - x y) from the
-// hardware's approximation of its leading bits: four FP64 instructions instead of seven.  The
-// residual of the last step is exact to far below an ulp, so the result is rounded once.
-__device__ __forceinline__ double rcp_newton(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
-}
-
-// a / b for b > 0: the quotient with the Newton reciprocal, corrected by its exact remainder (seven
-// FP64 instructions instead of ten); the plain division where the approximation would flush b
-__device__ __forceinline__ double quotient(double a, double b) {
-  if (dbits(b) < 0x0060000000000000LL) return a / b;
-  const double y = rcp_newton(b), q = a * y;
-  return fma(fma(-b, q, a), y, q);
-}
-
-// sqrt(x) for x > 0 by Goldschmidt's iteration from the hardware's approximation of 1 / sqrt(x), the last
-// step from the exact remainder x - g^2 (Markstein): six FP64 instructions instead of eleven; the
-// plain function outside the range where every intermediate is normal
-__device__ __forceinline__ double root(double x) {
-  if ((unsigned long long)(dbits(x) - 0x1000000000000000LL) > 0x6000000000000000ULL - 0x1000000000000000ULL) return sqrt(x);
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double h = __longlong_as_double(dbits(y) - (1LL << 52)), g = x * y;  // y / 2
-  const double r = fma(-g, h, 0.5);
-  g = fma(g, r, g);
-  h = fma(h, r, h);
-  return fma(fma(-g, g, x), h, g);
-}
-
 __device__ __forceinline__ double sound(double Tt) { return root(Tt * (5.0 / 6.0)); }
-
-// Viscosity mu0 T^omega about the cell's anchor v = (1 / T0, mu0 T0^omega in two words), 1 / T0 a float so
-// that x = T / T0 - 1 is rounded once: with |x| < 1/32 the binomial series of (1 + x)^omega - 1 takes
-// twelve FP64 instructions instead of the 53 of exp(omega log T) and the 120 or so of pow, and its error
-// is that of the anchor's power and of the last rounding, as for the product before.  A cell whose
-// temperature has left that range (at the first step 1 / T0 = 0) gets a new anchor by `power(T, e)`.
-template <typename Power>
-__device__ __forceinline__ double viscosity(double T, double mu0, double omega, const double *series, double *v, Power power) {
-  double x = fma(T, v[0], -1.0), hi = v[1], lo = v[2];
-  constexpr long long kSmall = 0x3fa0000000000000LL;  // 1/32
-  if ((dbits(x) & 0x7fffffffffffffffLL) >= kSmall) {
-    const double i0 = (double)(float)(1.0 / T), p = power(i0, -omega);
-    hi = mu0 * p;
-    lo = fma(mu0, p, -hi);
-    x = fma(T, i0, -1.0);
-    v[0] = i0;
-    v[1] = hi;
-    v[2] = lo;
-    if ((dbits(x) & 0x7fffffffffffffffLL) >= kSmall) {  // 1 / T is no float
-      v[0] = 0.0;
-      return mu0 * power(T, omega);
-    }
-  }
-  double s = series[MACRO_MU_SERIES - 1];
-#pragma unroll
-  for (int n = MACRO_MU_SERIES - 2; n >= 0; --n) s = fma(s, x, series[n]);
-  return hi + fma(hi, s * x, lo);
-}
 
 // A value with the number of the pass that wrote it, one 16-byte access (a single copy)
 __device__ __forceinline__ void st_tagged(double *p, double v, unsigned long long tag) {
