@@ -45,15 +45,14 @@ __device__ __forceinline__ double root(double x) {
 }
 
 // Viscosity mu0 T^omega about the cell's anchor v = (1 / T0, mu0 T0^omega in two words), 1 / T0 a float so
-// that x = T / T0 - 1 is rounded once: with |x| < 1/32 the binomial series of (1 + x)^omega - 1
+// that x = T / T0 - 1 is rounded once: inside the series' range the binomial series of (1 + x)^omega - 1
 // takes twelve FP64 instructions where the power takes a logarithm and an exponential, and its error is
 // that of the anchor's power and of the last rounding, as for the product before.  A cell whose
 // temperature has left that range (at the first step 1 / T0 = 0) gets a new anchor by `power(T, e)`.
 template <typename Power>
-__device__ __forceinline__ double viscosity(double T, double mu0, double omega, const double *series, double *v, Power power) {
+__device__ __forceinline__ double viscosity(double T, double mu0, double omega, const MuSeries &series, double *v, Power power) {
   double x = fma(T, v[0], -1.0), hi = v[1], lo = v[2];
-  constexpr long long kSmall = 0x3fa0000000000000LL;  // 1/32
-  if ((dbits(x) & 0x7fffffffffffffffLL) >= kSmall) {
+  if ((dbits(x) & 0x7fffffffffffffffLL) >= series.range) {
     const double i0 = (double)(float)(1.0 / T), p = power(i0, -omega);
     hi = mu0 * p;
     lo = fma(mu0, p, -hi);
@@ -61,14 +60,14 @@ __device__ __forceinline__ double viscosity(double T, double mu0, double omega, 
     v[0] = i0;
     v[1] = hi;
     v[2] = lo;
-    if ((dbits(x) & 0x7fffffffffffffffLL) >= kSmall) {  // 1 / T is no float
+    if ((dbits(x) & 0x7fffffffffffffffLL) >= series.range) {  // 1 / T is no float, or there is no range
       v[0] = 0.0;
       return mu0 * power(T, omega);
     }
   }
-  double s = series[MACRO_MU_SERIES - 1];
+  double s = series.c[MACRO_MU_SERIES - 1];
 #pragma unroll
-  for (int n = MACRO_MU_SERIES - 2; n >= 0; --n) s = fma(s, x, series[n]);
+  for (int n = MACRO_MU_SERIES - 2; n >= 0; --n) s = fma(s, x, series.c[n]);
   return hi + fma(hi, s * x, lo);
 }
 }  // namespace

@@ -322,8 +322,7 @@ struct gsis_solver {
   // Shakhov: A_tt = 2/3, no kr
   template <typename Args>
   void transport_coefficients(Args &m) const {
-    double b = 1.0;
-    for (int n = 0; n < MACRO_MU_SERIES; ++n) m.mu_series[n] = b = b * (omega - n) / (n + 1);
+    m.mu_series = viscosity_series(omega);
     m.vis = m_vis;
     m.kt_of_mu = 15.0 / 8.0;
     m.kr_of_mu = 0.0;

@@ -1,6 +1,7 @@
 // gsis_internal.h -- structures shared by the host solver object and the CUDA kernels.
 // Not part of the public ABI (include/gsis.h is).
 #pragma once
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -327,7 +328,27 @@ struct WallLoadArgs {
 };
 cudaError_t launch_wall_loads(const WallLoadArgs &a, cudaStream_t s);
 
-constexpr int MACRO_MU_SERIES = 9;  // terms of (1 + x)^omega - 1, |x| < 1/32: the next is below 2^-56
+// The viscosity's series (1 + x)^omega - 1 = sum_n (omega, n) x^n: its first terms, and the range of |x|
+// (as the bits of a double) where they suffice.  That is 1/32 while the next term is then at most 2^-56, as
+// for every omega in [0, 1] (|(omega, 10)| < 2^-6); else a smaller power of two, also such that the terms
+// fall, and 0 (never the series) where 2^-20 is not small enough.
+constexpr int MACRO_MU_SERIES = 9;
+struct MuSeries {
+  double c[MACRO_MU_SERIES];  // binomial coefficients (omega, n), n = 1, 2, ...
+  long long range;
+};
+inline MuSeries viscosity_series(double omega) {
+  MuSeries m{};
+  double b = 1.0;
+  for (int n = 0; n < MACRO_MU_SERIES; ++n) m.c[n] = b = b * (omega - n) / (n + 1);
+  const double next = std::fabs(b * (omega - MACRO_MU_SERIES) / (MACRO_MU_SERIES + 1));
+  for (int e = -5; e >= -20; --e)
+    if (std::ldexp(next, e * (MACRO_MU_SERIES + 1)) <= std::ldexp(1.0, -56) && std::fabs(omega) <= std::ldexp(1.0, -e)) {
+      m.range = (long long)(1023 + e) << 52;  // 2^e
+      break;
+    }
+  return m;
+}
 struct MacroArgs {
   KinGeom g;
   const AxisCell<double> *ax[3];
@@ -337,7 +358,7 @@ struct MacroArgs {
   double d_r, Z_r;
   double kt_of_mu, kr_of_mu;  // conductivities per viscosity (Eq. mu_kappa)
   double four_over_dr;        // 4 / d_r
-  double mu_series[MACRO_MU_SERIES];  // binomial coefficients (omega, n), n = 1, 2, ...
+  MuSeries mu_series;
   double *vis;                // [cell][3] the viscosity's anchor (work)
   double mass_ref;
   double den_floor;        // 1e-24 x total volume: fields with sum W_k^2 V below it count as zero
@@ -380,7 +401,7 @@ struct MacroGenArgs {
   double mu0, omega, cfl, tol, d_r, Z_r, mass_ref;
   double kt_of_mu, kr_of_mu;   // conductivities per viscosity (Eq. mu_kappa)
   double four_over_dr;         // 4 / d_r (Rykov)
-  double mu_series[MACRO_MU_SERIES];  // binomial coefficients (omega, n), n = 1, 2, ...
+  MuSeries mu_series;
   double *vis;                 // [cell][3] the viscosity's anchor (work)
   double vsum;                 // total volume (fields with sum W_k^2 V <= 1e-24 vsum count as zero)
   const GenCell<double> *gen;  // [cell] FP64 geometry

@@ -1,4 +1,5 @@
-"""The FP64 reciprocal, quotient and square root of the solver's kernels against CUDA's correctly rounded ones.
+"""The FP64 reciprocal, quotient and square root of the solver's kernels against CUDA's correctly rounded ones, and
+the viscosity's series against the power in quadruple or extended precision.
 
 Each ends in one rounding of a value that is exact to about 2^-80 (the residual of the last Newton step, or the
 exact remainder), so a result can differ from the correctly rounded one only where the exact value lies that
@@ -36,6 +37,7 @@ def probe(tmp_path_factory):
         assert lib.fp64_probe(which, len(x), ptr(x), ptr(y), ptr(own), ptr(ref)) == 0
         return own, ref
 
+    run.lib = lib
     return run
 
 
@@ -95,3 +97,33 @@ def test_limiter_of_tails_below_the_normal_numbers():
     scaled_close(g.W(), o.W(), 1e-10, "W with a vanishing limiter constant")
     assert np.isfinite(g.get_f()).all()
     g.close()
+
+
+# Bound, in 2^-53: CUDA's pow 2 ulp (4), the anchor's product and the last addition 1 each, the series at most six
+# roundings of a sum that is at most e - 1 times the result (12), what it leaves out 2^-3 and a fall of the
+# later terms by at most 1/2 each: 20 in all.
+@pytest.mark.parametrize("omega", [0.0, 0.5, 0.74, 0.81, 1.0, 1.5, -0.5, -3.0, 6.5, 12.0, 30.0, -40.0, 1e4, 3e7])
+def test_viscosity_for_any_exponent(probe, omega):
+    rng = np.random.default_rng(4)
+    n = 1 << 18
+    span = min(1.0, 300.0 / max(abs(omega), 1e-9))  # |log T| of the anchors: T^omega stays in range
+    T0 = np.exp(rng.uniform(-span, span, n))
+    x = np.where(np.arange(n) % 4 == 0, rng.uniform(-0.5, 0.5, n), rng.uniform(-1.0, 1.0, n) * 2.0 ** -rng.integers(5, 24, n))
+    T = T0 * (1.0 + (x if abs(omega) <= 40.0 else x / abs(omega)))
+    own, ref = np.empty(n), np.empty(n)
+    mu0 = 0.0564
+    ptr = lambda a: a.ctypes.data_as(C.c_void_p)  # noqa: E731
+    assert probe.lib.fp64_probe_viscosity(C.c_double(mu0), C.c_double(omega), n, ptr(T), ptr(T0), ptr(own), ptr(ref)) == 0
+    for got, at, what in ((ref, T0, "the anchor"), (own, T, "its neighbourhood")):
+        want = np.longdouble(mu0) * np.power(at.astype(np.longdouble), np.longdouble(omega))
+        err = float((np.abs(got - want) / want).max())
+        assert err <= 20 * 2.0 ** -53, f"omega {omega}: {err * 2.0 ** 53:.1f} x 2^-53 off at {what}"
+
+
+@pytest.mark.parametrize("omega", [np.nan, np.inf])
+def test_viscosity_of_no_number(probe, omega):
+    T = np.array([0.5, 1.0, 2.0])
+    own, ref = np.empty(3), np.empty(3)
+    ptr = lambda a: a.ctypes.data_as(C.c_void_p)  # noqa: E731
+    assert probe.lib.fp64_probe_viscosity(C.c_double(1.0), C.c_double(omega), 3, ptr(T), ptr(T), ptr(own), ptr(ref)) == 0
+    assert np.array_equal(own, np.power(T, omega), equal_nan=True) and np.array_equal(ref, own, equal_nan=True)
