@@ -1960,10 +1960,10 @@ static int allocate_and_upload(gsis_solver *s) {
 #define A(ptr, bytes) \
   if (!rc) rc = s->alloc(&(ptr), (bytes))
   A(s->d_f, (size_t)s->nvdf * s->nslots * nc * sizeof(S));
-  // moment chunks: enough (cell, chunk) threads to fill the GPU, at most 64 blocks per chunk
+  // moment chunks: enough (cell, chunk) threads to fill the GPU, at most MOM_MAX_BLOCKS blocks per chunk
   {
     const int want = std::max(1, (int)((160000 + nc - 1) / nc));
-    s->mom_bpc = std::max(1, std::min(64, (s->nblocks + want - 1) / want));
+    s->mom_bpc = std::max(1, std::min(MOM_MAX_BLOCKS, (s->nblocks + want - 1) / want));
     s->mom_nchunks = (s->nblocks + s->mom_bpc - 1) / s->mom_bpc;
   }
   s->origin_mom = std::is_same<T, double>::value && s->nvdf == 1 && !s->point_set;

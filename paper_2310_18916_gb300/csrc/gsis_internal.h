@@ -195,6 +195,7 @@ size_t kinetic_gscratch_stride(const KinGeom &g, int nvdf);
 template <typename T, typename S>
 cudaError_t launch_wall_prepass(const KinArgs<T, S> &a, const int *wall_cell, const int *wall_side, int nwall,
                                 const double *Z0, double *rho_w, int nslots, cudaStream_t s);
+constexpr int MOM_MAX_BLOCKS = 64;  // velocity blocks of a moment chunk at most
 template <typename T, typename S>
 cudaError_t launch_moments(const KinArgs<T, S> &a, int blocks_per_chunk, int nchunks, double *mp, cudaStream_t s);
 // FP64 storage on a tensor-product grid, Shakhov: moments about the origin into chunks 0..nchunks-1 of mp,

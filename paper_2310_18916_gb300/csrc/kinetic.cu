@@ -539,7 +539,13 @@ cudaError_t kinetic_shape(const KinGeom &g, int nvdf, bool gm, bool fx, int want
   cudaError_t e = cudaFuncGetAttributes(&attr, k);
   if (e != cudaSuccess) return e;
   *warps = std::max(1, std::min(want_warps, attr.maxThreadsPerBlock / 32));
-  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the limit belongs to the kernel and all host threads' solvers launch it: always what the device
+  // allows, never what one solver needs
+  int dev = 0, optin = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)attr.sharedSizeBytes);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, k, *warps * 32, smem);
 }
@@ -547,8 +553,6 @@ cudaError_t kinetic_shape(const KinGeom &g, int nvdf, bool gm, bool fx, int want
 template <typename T, typename S>
 cudaError_t launch_kinetic(const KinArgs<T, S> &a, int nblocks, int nwarps, size_t smem, cudaStream_t s) {
   void (*k)(const KinArgs<T, S>) = kinetic_fn<T, S>(a.g, a.nvdf, a.gscratch != nullptr, a.ftab != nullptr);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   k<<<nblocks, nwarps * 32, smem, s>>>(a);
   return cudaGetLastError();
 }
@@ -865,7 +869,8 @@ template <typename T, typename S>
 cudaError_t launch_moments(const KinArgs<T, S> &a, int blocks_per_chunk, int nchunks, double *mp, cudaStream_t s) {
   const size_t smem = (size_t)blocks_per_chunk * VB * 4 * sizeof(T);
   auto k = a.nvdf == 2 ? moments_kernel<T, S, 2> : moments_kernel<T, S, 1>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (the same limit for every solver: see kinetic_shape)
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, MOM_MAX_BLOCKS * VB * 4 * (int)sizeof(T));
   if (e != cudaSuccess) return e;
   dim3 grid((a.g.nc + 127) / 128, nchunks);
   k<<<grid, 128, smem, s>>>(a, blocks_per_chunk, mp);
