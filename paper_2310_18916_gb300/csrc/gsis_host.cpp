@@ -258,6 +258,9 @@ struct gsis_solver {
     allocs.clear();
   }
 
+  // whether steps or presteps of this solver run the synthetic solve
+  bool synthetic() const { return opt.mode == GSIS_MODE_GSIS || opt.euler_presteps > 0; }
+
   int cuda(cudaError_t e, const char *what) {
     if (e == cudaSuccess) return GSIS_OK;
     return fail(GSIS_E_CUDA, "%s: %s", what, cudaGetErrorString(e));
@@ -341,7 +344,6 @@ struct gsis_solver {
     MacroGenArgs m{};
     m.nc = (int)nc;
     m.nW = gas.model == GSIS_RYKOV ? 6 : 5;
-    m.model = gas.model;
     m.steps = opt.macro_steps;
     m.sweeps = opt.macro_sweeps;
     m.closed = closed;
@@ -573,7 +575,6 @@ struct gsis_solver {
       m.omega = omega;
       m.cfl = opt.macro_cfl;
       m.tol = opt.macro_tol;
-      m.model = gas.model;
       m.nW = gas.model == GSIS_RYKOV ? 6 : 5;
       m.steps = opt.macro_steps;
       m.sweeps = opt.macro_sweeps;
@@ -1639,7 +1640,7 @@ static int setup_velocities(gsis_solver *s, const gsis_vgrid *vg);
 static int setup(gsis_solver *s, const gsis_mesh *m, const gsis_vgrid *vg) {
   int rc0 = m->ncells > 0 ? setup_unstructured_mesh(s, m) : setup_mesh(s, m);
   if (rc0) return rc0;
-  if (s->general && (s->opt.mode == GSIS_MODE_GSIS || s->opt.euler_presteps > 0)) macro_general_faces(s);
+  if (s->general && s->synthetic()) macro_general_faces(s);
   return setup_velocities(s, vg);
 }
 
@@ -1832,6 +1833,11 @@ static int setup_velocities(gsis_solver *s, const gsis_vgrid *vg) {
 // placement follows the shared-memory limit of the sm_100 family, 227 KB.
 template <typename T, typename S>
 static int plan_kinetic(gsis_solver *s) {
+  // moment chunks: enough (cell, chunk) threads to fill the GPU, at most MOM_MAX_BLOCKS blocks per chunk
+  const int want_chunks = std::max(1, (int)((160000 + (size_t)s->nc - 1) / s->nc));
+  s->mom_bpc = std::max(1, std::min(MOM_MAX_BLOCKS, (s->nblocks + want_chunks - 1) / want_chunks));
+  s->mom_nchunks = (s->nblocks + s->mom_bpc - 1) / s->mom_bpc;
+  s->origin_mom = std::is_same<T, double>::value && s->nvdf == 1 && !s->point_set;
   if (s->general) {
     int dev = 0, sms = 152;
     const bool have_dev = cudaGetDevice(&dev) == cudaSuccess &&
@@ -1890,31 +1896,6 @@ static int plan_kinetic(gsis_solver *s) {
   return GSIS_OK;
 }
 
-static size_t footprint(const gsis_solver *s) {
-  const size_t T = s->prec == GSIS_F64 ? 8 : 4;                             // kinetic arithmetic
-  const size_t Sb = s->prec == GSIS_F64 ? 8 : (s->prec == GSIS_BF16 ? 2 : 4);  // VDF storage
-  const size_t nc = s->nc;
-  size_t b = 0;
-  b += (size_t)s->nvdf * s->nslots * nc * Sb;  // f (f0, f1)
-  b += (size_t)s->nblocks * (s->nwall + 1) * NWF * T;  // wall partials
-  b += s->kin_scratch_bytes;                          // kinetic ring or work arrays in global memory
-  if (s->general) b += nc * (sizeof(GenCell<double>) + sizeof(GenRec<double>) + 6 * (2 * sizeof(int) + 1)) + s->units.size() * sizeof(int2) + (size_t)s->nwall * 8;
-  if (s->unstructured) b += 14 * nc + (nc + 1) * 4 + s->gs_idx.size() * (4 + 3 * (T + 8));
-  if (s->general && (s->opt.mode == GSIS_MODE_GSIS || s->opt.euler_presteps > 0))
-    b += nc * (sizeof(GenCell<double>) + (3 + 6 * (size_t)s->kin_grid + 6 + 6 + 4 + 18 + 15 + 6 + 6 + 6 + 36 + 6 + 6 + 6 + 6 + 18 + 72) * 8 + 13 * 4);
-  b += (size_t)nc * moment_len(s->nvdf) * 8 * 16;  // moment chunks (bounded)
-  if (s->factored)  // one-dimensional Maxwellian factors
-    b += nc * (s->vaxis.size() / 2) * factor_table_len(s->nvdf) * 8 + (size_t)s->nslots * 4 + s->vaxis.size() * 8;
-  if (!s->general) b += nc * T;
-  if (Sb == 8 && s->nvdf == 1 && !s->point_set)  // FP64 origin moments: the extra chunk, the table
-    b += (size_t)nc * moment_len(1) * 8 + (size_t)s->nslots * 16 * 8 + s->vaxis.size() * 8;
-  b += nc * NST * (T + 8);                    // states
-  b += nc * (13 + 18 + 18 + 12 + 6 + 6 + 1) * 8;
-  b += nc * (6 + 6 + 18 + 15 + 4 + 6 + 2 + 1 + 18 + 6 + 3 + 18 + 72) * 8 + nc * 4;  // synthetic-solve work
-  b += (size_t)s->nslots * 4 * (T + 8) + (size_t)s->nwall * 32 * 8 + 3 * nc * 4 + (1 << 20);
-  return b;
-}
-
 // the kinetic kernel's per-cell records
 template <typename T>
 static std::vector<GenRec<T>> gen_records(const gsis_solver *s) {
@@ -1953,20 +1934,12 @@ static std::vector<GenRec<T>> gen_records(const gsis_solver *s) {
   return out;
 }
 
-template <typename T, typename S>
-static int allocate_and_upload(gsis_solver *s) {
+// Every device array a solver holds, as each(pointer, bytes): gsis_create allocates from this list and
+// gsis_footprint_bytes adds it up.  (The arrays of a synthetic solve only where the solver runs it.)
+template <typename T, typename S, typename Each>
+static void device_arrays(gsis_solver *s, Each &&A) {
   const size_t nc = s->nc;
-  int rc = 0;
-#define A(ptr, bytes) \
-  if (!rc) rc = s->alloc(&(ptr), (bytes))
   A(s->d_f, (size_t)s->nvdf * s->nslots * nc * sizeof(S));
-  // moment chunks: enough (cell, chunk) threads to fill the GPU, at most MOM_MAX_BLOCKS blocks per chunk
-  {
-    const int want = std::max(1, (int)((160000 + nc - 1) / nc));
-    s->mom_bpc = std::max(1, std::min(MOM_MAX_BLOCKS, (s->nblocks + want - 1) / want));
-    s->mom_nchunks = (s->nblocks + s->mom_bpc - 1) / s->mom_bpc;
-  }
-  s->origin_mom = std::is_same<T, double>::value && s->nvdf == 1 && !s->point_set;
   A(s->d_mp, (size_t)(s->mom_nchunks + (s->origin_mom ? 1 : 0)) * nc * moment_len(s->nvdf) * sizeof(double));
   const bool tiled = s->kg.tile[0] > 0;
   const int tile_nodes = s->kg.tile[0] + s->kg.tile[1] + s->kg.tile[2];
@@ -1988,7 +1961,7 @@ static int allocate_and_upload(gsis_solver *s) {
     A(s->d_gin, 6 * nc);
     A(s->d_wall_area, (size_t)(s->nwall + 1) * sizeof(double));
     A(s->d_wden, (size_t)(s->nwall + 1) * sizeof(double));
-    if (s->opt.mode == GSIS_MODE_GSIS || s->opt.euler_presteps > 0) {
+    if (s->synthetic()) {
       A(s->d_gen64, nc * sizeof(GenCell<double>));
       A(s->d_xc, 3 * nc * sizeof(double));
       A(s->d_kpart, (size_t)s->kin_grid * nc * 6 * sizeof(double));
@@ -2055,37 +2028,49 @@ static int allocate_and_upload(gsis_solver *s) {
   A(s->d_ticket, 4 * sizeof(unsigned));
   A(s->d_bar, MACRO_BAR_WORDS * sizeof(unsigned));
   A(s->d_err, sizeof(int));
+  A(s->d_iters, sizeof(int));
+  if (s->synthetic()) {
+    A(s->d_colcells, nc * sizeof(int));
+    A(s->m_vis, nc * 3 * sizeof(double));
+    A(s->m_red, ((size_t)3 * MACRO_MAX_GRID * 16 + 32) * sizeof(double));
+  }
+  if (s->synthetic() && !s->general) {
+    A(s->m_W, nc * 6 * sizeof(double));
+    A(s->m_pr, nc * 6 * sizeof(double));
+    A(s->m_gW, nc * 18 * sizeof(double));
+    A(s->m_gP, nc * 15 * sizeof(double));
+    A(s->m_aux, nc * 4 * sizeof(double));
+    A(s->m_R, nc * 6 * sizeof(double));
+    A(s->m_invD, nc * 2 * sizeof(double));
+    A(s->d_ivol, nc * sizeof(double));
+    A(s->m_Fc, nc * 18 * sizeof(double));
+    A(s->m_corr, nc * 6 * sizeof(double));
+    A(s->m_gam, nc * 3 * sizeof(double));
+    A(s->m_Ffc, nc * 36 * sizeof(double));
+    A(s->m_G, nc * 72 * sizeof(double));
+    A(s->d_colnat, nc * sizeof(int));
+    A(s->m_wfl, (size_t)(s->nwall + 1) * 6 * sizeof(double));
+  }
+}
+
+template <typename T, typename S>
+static int allocate_and_upload(gsis_solver *s) {
+  const size_t nc = s->nc;
+  int rc = 0;
+  device_arrays<T, S>(s, [&](auto &ptr, size_t bytes) {
+    if (!rc) rc = s->alloc(&ptr, bytes);
+  });
   if (!rc && cudaHostAlloc((void **)&s->pin, sizeof(gsis_solver::Readback), cudaHostAllocDefault) != cudaSuccess)
     rc = s->fail(GSIS_E_OOM, "pinned host read-back words");
-  A(s->d_iters, sizeof(int));
-  A(s->m_W, nc * 6 * sizeof(double));
-  A(s->m_pr, nc * 6 * sizeof(double));
-  A(s->m_gW, nc * 18 * sizeof(double));
-  A(s->m_gP, nc * 15 * sizeof(double));
-  A(s->m_aux, nc * 4 * sizeof(double));
-  A(s->d_colcells, nc * sizeof(int));
-  A(s->m_R, nc * 6 * sizeof(double));
-  A(s->m_invD, nc * 2 * sizeof(double));
-  A(s->d_ivol, nc * sizeof(double));
-  A(s->m_Fc, nc * 18 * sizeof(double));
-  A(s->m_corr, nc * 6 * sizeof(double));
-  A(s->m_gam, nc * 3 * sizeof(double));
-  A(s->m_Ffc, nc * 36 * sizeof(double));
-  A(s->m_vis, nc * 3 * sizeof(double));
-  A(s->m_G, nc * 72 * sizeof(double));
-  A(s->d_colnat, nc * sizeof(int));
-  A(s->m_wfl, (size_t)(s->nwall + 1) * 6 * sizeof(double));
-#undef A
   if (rc) return rc;
   rc = s->cuda(macro_launch_shape((int)nc, s->opt.macro_sms, &s->macro_grid, &s->macro_block), "occupancy");
-  if (rc) return rc;
-  rc = s->alloc(&s->m_red, ((size_t)3 * s->macro_grid * 16 + 32) * sizeof(double));
   if (rc) return rc;
   std::vector<T> velT(s->vel64.begin(), s->vel64.end());
   rc = s->upload(s->d_vel, velT.data(), velT.size() * sizeof(T));
   std::vector<double> mtab;
   if (s->origin_mom) {
-    if (tiled) {
+    if (s->kg.tile[0] > 0) {
+      const int tile_nodes = s->kg.tile[0] + s->kg.tile[1] + s->kg.tile[2];
       // per block and node of its tile on each axis: w, w xi, w xi^2, w xi^3 of that axis
       mtab.assign((size_t)s->nblocks * tile_nodes * 4, 0.0);
       const int nx = s->nv_axis[0], ny = s->nv_axis[1], nn = nx + ny + s->nv_axis[2];
@@ -2171,19 +2156,18 @@ static int allocate_and_upload(gsis_solver *s) {
   if (!rc) rc = s->upload(s->d_wall_uT, uT, sizeof uT);
   if (!rc) rc = s->cuda(cudaStreamSynchronize(s->stream), "sync");  // uT leaves scope
   if (!rc) rc = s->upload(s->d_vol, s->vol.data(), nc * sizeof(double));
-  std::vector<double> ivol(nc);
-  for (size_t c = 0; c < nc; ++c) ivol[c] = 1.0 / s->vol[c];
-  if (!rc) rc = s->upload(s->d_ivol, ivol.data(), nc * sizeof(double));
-  if (!rc) rc = s->cuda(cudaStreamSynchronize(s->stream), "sync");  // ivol leaves scope
-  if (!rc) rc = s->upload(s->d_colcells, s->colcells.data(), nc * sizeof(int));
-  std::vector<int> colnat(s->general ? 0 : nc);
-  for (size_t e = 0; e < colnat.size(); ++e) {
-    const int c = s->colcells[e];
-    colnat[e] = c % s->n[0] | (c / s->n[0]) % s->n[1] << 10 | c / (s->n[0] * s->n[1]) << 20;
-  }
-  if (!rc && !colnat.empty()) {
-    rc = s->upload(s->d_colnat, colnat.data(), nc * sizeof(int));
-    if (!rc) rc = s->cuda(cudaStreamSynchronize(s->stream), "sync");  // colnat leaves scope
+  if (!rc && s->d_colcells) rc = s->upload(s->d_colcells, s->colcells.data(), nc * sizeof(int));
+  if (!rc && s->d_colnat) {
+    std::vector<double> ivol(nc);
+    std::vector<int> colnat(nc);
+    for (size_t e = 0; e < nc; ++e) {
+      const int c = s->colcells[e];
+      ivol[e] = 1.0 / s->vol[e];
+      colnat[e] = c % s->n[0] | (c / s->n[0]) % s->n[1] << 10 | c / (s->n[0] * s->n[1]) << 20;
+    }
+    rc = s->upload(s->d_ivol, ivol.data(), nc * sizeof(double));
+    if (!rc) rc = s->upload(s->d_colnat, colnat.data(), nc * sizeof(int));
+    if (!rc) rc = s->cuda(cudaStreamSynchronize(s->stream), "sync");  // ivol and colnat leave scope
   }
   if (!rc && s->general) {
     const std::vector<GenCell<T>> gT = cast_gen<T>(s->gen64);
@@ -2208,6 +2192,7 @@ static int allocate_and_upload(gsis_solver *s) {
       if (!rc) rc = s->upload(s->d_cmask, s->cmask.data(), nc * sizeof(int));
       if (!rc) rc = s->upload(s->d_faces, s->faces.data(), s->faces.size() * sizeof(int));
     }
+    if (!rc) rc = s->cuda(cudaStreamSynchronize(s->stream), "sync");  // gT and recs leave scope
   }
   if (!rc) rc = s->cuda(cudaMemsetAsync(s->d_ticket, 0, 4 * sizeof(unsigned), s->stream), "memset");
   if (!rc) rc = s->cuda(cudaMemsetAsync(s->d_err, 0, sizeof(int), s->stream), "memset");
@@ -2241,7 +2226,9 @@ extern "C" int gsis_footprint_bytes(const gsis_mesh *mesh, const gsis_vgrid *vgr
   rc = setup(&tmp, mesh, vgrid);
   if (!rc) rc = GSIS_DISPATCH(tmp.prec, (plan_kinetic<T, S>(&tmp)));
   if (rc) return rc;
-  *bytes = footprint(&tmp);
+  size_t sum = 0;
+  GSIS_DISPATCH(tmp.prec, (device_arrays<T, S>(&tmp, [&](auto &, size_t b) { sum += b; }), 0));
+  *bytes = sum;
   return GSIS_OK;
 }
 

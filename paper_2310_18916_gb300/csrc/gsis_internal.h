@@ -243,7 +243,7 @@ cudaError_t kinetic_shape(const KinGeom &g, int nvdf, bool gm, bool fx, int want
                           int *ctas_per_sm);
 // the table of one-dimensional Maxwellian factors of the current state (KinArgs::ftab); values per
 // node, and the launch (nodes of x, y, z in vaxis)
-constexpr int factor_table_len(int nvdf) { return nvdf == 2 ? 8 : 4; }
+__host__ __device__ constexpr int factor_table_len(int nvdf) { return nvdf == 2 ? 8 : 4; }
 cudaError_t launch_factor_table(int nc, const int *nv_axis, int nvdf, const double *st64, const double *vaxis, double *tab,
                                 cudaStream_t s);
 
@@ -355,7 +355,7 @@ struct MacroArgs {
   const AxisCell<double> *ax[3];
   double Kn, omega, cfl, tol;
   double mu0;              // Kn / sqrt(pi): mu = mu0 T^omega
-  int model, nW, steps, sweeps;
+  int nW, steps, sweeps;
   double d_r, Z_r;
   double kt_of_mu, kr_of_mu;  // conductivities per viscosity (Eq. mu_kappa)
   double four_over_dr;        // 4 / d_r
@@ -386,7 +386,7 @@ struct MacroArgs {
 // The synthetic solve on general meshes (one cooperative kernel, macro_general.cu)
 constexpr int MACRO_MAX_COLOURS = 32;  // colours of the synthetic solve's sweeps at most
 struct MacroGenArgs {
-  int nc, nW, model, steps, sweeps, closed;
+  int nc, nW, steps, sweeps, closed;
   int flat;                    // no face normal and no gradient weight has a z component (up to rounding)
   int layer;                   // sides 4 and 5 of the cells carry no flux
   int ncolm;                   // colours of the LU-SGS passes (cells of colour k: colcells[colm_off[k] ..])

@@ -115,8 +115,6 @@ struct KinSmem {
 // FP64 pipe's rate: 128^2 cells with 32^3 velocities 115.1 -> 62.7 ms (floor of those instructions
 // 57), the wall pre-pass 4.2 -> 1.1; Rykov 48^2 with 20^3 10.9 -> 5.2.  FP32 keeps its exponentials
 // (MUFU), cheaper there than gathered factors.
-constexpr int FT_SHAKHOV = 4, FT_RYKOV = 8;
-__host__ __device__ constexpr int factor_len(int nvdf) { return nvdf == 2 ? FT_RYKOV : FT_SHAKHOV; }
 
 __global__ void __launch_bounds__(128) factor_table_kernel(int nc, int nx, int ny, int nz, int nvdf, const double *st64,
                                                            const double *vaxis, double *tab) {
@@ -128,7 +126,7 @@ __global__ void __launch_bounds__(128) factor_table_kernel(int nc, int nx, int n
     const int a = node < nx ? 0 : (node < nx + ny ? 1 : 2);
     const double *st = st64 + cell * NST;
     const double xi = vaxis[node], c = xi - st[a], co = xi - st[5 + a];
-    double *o = tab + i * factor_len(nvdf);
+    double *o = tab + i * factor_table_len(nvdf);
     double en = exp(-c * c * st[3]), eo = exp(-co * co * st[8]);
     if (a == 0) {
       en *= st[4];
@@ -162,7 +160,7 @@ cudaError_t launch_factor_table(int nc, const int *nv_axis, int nvdf, const doub
 template <int NV>
 __device__ __forceinline__ void corrected_factored(const double *stored, const double *row, const int *node, double s,
                                                    double cn, double co, double *f) {
-  constexpr int L = factor_len(NV);
+  constexpr int L = factor_table_len(NV);
   double2 e[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) e[a] = __ldg(reinterpret_cast<const double2 *>(row + node[a] * L));
@@ -216,7 +214,7 @@ __global__ void kinetic_kernel(const KinArgs<T, S> A) {
     node[1] = packed >> 10 & 1023;
     node[2] = packed >> 20;
   }
-  const unsigned frow = A.nnode * factor_len(NV);  // doubles per cell of the table
+  const unsigned frow = A.nnode * factor_table_len(NV);  // doubles per cell of the table
   const T e2 = (T)0.5 * (xi[0] * xi[0] + xi[1] * xi[1] + xi[2] * xi[2]);
   T axi[3], Mw[3], Mw1[3];
   int upside[3];
@@ -236,7 +234,6 @@ __global__ void kinetic_kernel(const KinArgs<T, S> A) {
   F[0] = A.f + (size_t)b * G.nc * VB;
   if constexpr (NV == 2) F[NV - 1] = A.f1 + (size_t)b * G.nc * VB;
   const int4 *natcell = A.natcell + (size_t)oct * G.nc;
-  const T K3 = (T)G.K3;
   const size_t slot_stride = (size_t)G.maxcol * NV * VB;
   const int tid = threadIdx.x, nthr = blockDim.x;
   // Colour c + 2's stored f rows (VB values per cell and VDF) and state rows are copied into the
@@ -410,7 +407,7 @@ __global__ void kinetic_kernel(const KinArgs<T, S> A) {
       T mw, g[NV];  // mw: Maxwellian of W^n
       if constexpr (FX) {
         const T *row = A.ftab + (size_t)(unsigned)cell * frow;
-        constexpr int FL = factor_len(NV);
+        constexpr int FL = factor_table_len(NV);
         T v[3][FL];
 #pragma unroll
         for (int a = 0; a < 3; ++a)
@@ -591,12 +588,12 @@ __global__ void wall_prepass_kernel(const KinArgs<T, S> A, const int *wall_cell,
   for (int a = 0; a < NACT; ++a) gc[a] = A.ax[a][nat[a]];
   const T eps2 = A.eps2[cell];
   // f^n of this thread's velocity in a cell (f0: the mass flux needs no other)
-  const unsigned frow = A.nnode * factor_len(A.nvdf);
+  const unsigned frow = A.nnode * factor_table_len(A.nvdf);
   auto value = [&](int c, const T *sc, size_t at, const T *v, const int *node) {
     const T raw = Fio<T, S>::ld(A.f + at);
     if constexpr (FX) {
       const T *row = A.ftab + (size_t)(unsigned)c * frow;
-      const int L = factor_len(A.nvdf);
+      const int L = factor_table_len(A.nvdf);
       double2 e[3];
 #pragma unroll
       for (int a = 0; a < 3; ++a) e[a] = __ldg(reinterpret_cast<const double2 *>(row + node[a] * L));

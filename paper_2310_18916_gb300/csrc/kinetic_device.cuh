@@ -145,9 +145,7 @@ __device__ __forceinline__ float smaller(float a, float b) { return a < b ? a : 
 // a > 0
 __device__ __forceinline__ bool is_positive(double a) { return __double_as_longlong(a) > 0; }
 __device__ __forceinline__ bool is_positive(float a) { return a > 0.f; }
-// a <= b and a < b for a, b >= 0 (non-negative doubles order like their bit patterns)
-__device__ __forceinline__ bool nonneg_le(double a, double b) { return __double_as_longlong(a) <= __double_as_longlong(b); }
-__device__ __forceinline__ bool nonneg_le(float a, float b) { return a <= b; }
+// a < b for a, b >= 0 (non-negative doubles order like their bit patterns)
 __device__ __forceinline__ bool nonneg_lt(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
 __device__ __forceinline__ bool nonneg_lt(float a, float b) { return a < b; }
 
@@ -232,24 +230,6 @@ __device__ __forceinline__ void load_state(const double *__restrict__ src, doubl
     st[2 * q] = v.x;
     st[2 * q + 1] = v.y;
   }
-}
-
-// Sum over the 32 lanes of v[0..31] by recursive halving: at each level a lane keeps the half
-// of its vector selected by one bit of its lane index and adds the partner's copy of that half.
-// Afterwards lane l holds the warp total of v[l] (31 shuffles instead of 5 per value).
-template <typename T>
-__device__ __forceinline__ T transpose_reduce(T *v, int lane) {
-#pragma unroll
-  for (int h = 16; h > 0; h >>= 1) {
-    const bool up = lane & h;
-#pragma unroll
-    for (int i = 0; i < h; ++i) {
-      const T send = up ? v[i] : v[i + h];
-      const T keep = up ? v[i + h] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
-    }
-  }
-  return v[0];
 }
 
 template <typename T>
