@@ -20,6 +20,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -49,8 +50,9 @@ MACRO_FLOPS_PER_CELL_STEP_2D = 1133
 # update and the published face increments 4.
 KINETIC_FLOPS_PER_POINT_2D = 64
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the 128^2 cavity with
-# 32^3 velocities, keyed by kernel, precision and the SHA-256 prefix of the kernel's source file
-# at capture time: a figure whose source has changed since is reported as null (stale).  Captured
+# 32^3 velocities, keyed by kernel, precision and the SHA-256 prefix of the kernel's sources (its file
+# and every header of the project that it includes) at capture time: a figure whose sources have
+# changed since is reported as null (stale).  Captured
 # on the 64^2 case in the same launch configuration as at 128^2 (FP64: the colour ring in device
 # scratch; FP32 and BF16: in shared memory) and scaled by the 4x cells: the kinetic kernel's
 # traffic is per point, the synthetic solve's per cell (profiles/dram_bytes_cavity64x32.md).
@@ -60,13 +62,28 @@ DRAM_BYTES_PER_LAUNCH = {
     ("kinetic_kernel", "bf16"): (4 * (0.2707e9 + 0.2125e9), "e82dbd7e9971"),
     ("macro_kernel", "f64"): (4 * (4.02e6 + 0.11e6), "3411d2b49067"),
 }
-KERNEL_SOURCES = {"kinetic_kernel": "kinetic.cu", "moments_kernel": "kinetic.cu", "macro_kernel": "macro.cu"}
+KERNEL_FILES = {"kinetic_kernel": "kinetic.cu", "macro_kernel": "macro.cu"}
+CSRC = os.path.join(ROOT, "paper_2310_18916_gb300", "csrc")
+
+
+def kernel_sources(kernel):
+    """The kernel's file and the project's headers it includes, directly or not, sorted by name."""
+    found, todo = set(), [KERNEL_FILES[kernel]]
+    while todo:
+        name = todo.pop()
+        if name not in found and os.path.exists(os.path.join(CSRC, name)):
+            found.add(name)
+            with open(os.path.join(CSRC, name)) as fh:
+                todo += re.findall(r'^\s*#include "([^"]+)"', fh.read(), flags=re.M)
+    return sorted(found)
 
 
 def source_sha(kernel):
-    path = os.path.join(ROOT, "paper_2310_18916_gb300", "csrc", KERNEL_SOURCES[kernel])
-    with open(path, "rb") as fh:
-        return hashlib.sha256(fh.read()).hexdigest()[:12]
+    h = hashlib.sha256()
+    for name in kernel_sources(kernel):
+        with open(os.path.join(CSRC, name), "rb") as fh:
+            h.update(name.encode() + b"\0" + fh.read())
+    return h.hexdigest()[:12]
 
 
 def traffic(kernel, precision):
