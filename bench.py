@@ -57,10 +57,10 @@ KINETIC_FLOPS_PER_POINT_2D = 64
 # scratch; FP32 and BF16: in shared memory) and scaled by the 4x cells: the kinetic kernel's
 # traffic is per point, the synthetic solve's per cell (profiles/dram_bytes_cavity64x32.md).
 DRAM_BYTES_PER_LAUNCH = {
-    ("kinetic_kernel", "f64"): (4 * (1.1842e9 + 1.3578e9), "e82dbd7e9971"),
-    ("kinetic_kernel", "f32"): (4 * (0.5406e9 + 0.4760e9), "e82dbd7e9971"),
-    ("kinetic_kernel", "bf16"): (4 * (0.2707e9 + 0.2125e9), "e82dbd7e9971"),
-    ("macro_kernel", "f64"): (4 * (4.02e6 + 0.11e6), "3411d2b49067"),
+    ("kinetic_kernel", "f64"): (4 * (1.1846e9 + 1.3590e9), "5a22bd081cf3"),
+    ("kinetic_kernel", "f32"): (4 * (0.5408e9 + 0.4760e9), "5a22bd081cf3"),
+    ("kinetic_kernel", "bf16"): (4 * (0.2707e9 + 0.2125e9), "5a22bd081cf3"),
+    ("macro_kernel", "f64"): (4 * (4.21e6 + 0.07e6), "b6173e018c54"),
 }
 KERNEL_FILES = {"kinetic_kernel": "kinetic.cu", "macro_kernel": "macro.cu"}
 CSRC = os.path.join(ROOT, "paper_2310_18916_gb300", "csrc")

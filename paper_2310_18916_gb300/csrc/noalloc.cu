@@ -62,8 +62,11 @@ struct Comp {
 // of the cell's row); lane partials are reduced over the warp in FP64 in a fixed order.
 // What bounds it: with one velocity's loads in flight per lane, their latency; the sums' order is the
 // same with kAhead of them.  9100 cells x 24^3: 1 / 4 / 8 / 16 in flight 590 / 614 / 497 / 557 us (16
-// leaves too few warps); left is the issue of the compensated sums, about 85 FP32 instructions per
-// 32 points.
+// leaves too few warps), 9100 x 20^3 486 / - / 425 / -.  A chunk of fewer than 32 kAhead velocities goes
+// through the loop of one alone, so nothing changes with fewer than about 740 cells at 24^3 or 6700 at 12^3
+// (500 x 24^3 411 / 410, 9100 x 12^3 389 / 389).  The issue of the compensated sums, about 85 FP32
+// instructions per 32 points, is 55 % of the 497 us; the rest is the loads, 16 B of velocity for
+// every 4 B of f in each of the two passes.
 // PASS 1 sums w f (1, xi); PASS 2 sums w f (c, cc, |c|^2 c) with c = xi - d, d read from
 // out[cell][1..3] where pass 1's reduction left it.
 template <int PASS>
