@@ -2029,28 +2029,31 @@ static void device_arrays(gsis_solver *s, Each &&A) {
   A(s->d_bar, MACRO_BAR_WORDS * sizeof(unsigned));
   A(s->d_err, sizeof(int));
   A(s->d_iters, sizeof(int));
-  if (s->synthetic()) {
-    A(s->d_colcells, nc * sizeof(int));
-    A(s->m_vis, nc * 3 * sizeof(double));
-    A(s->m_red, ((size_t)3 * MACRO_MAX_GRID * 16 + 32) * sizeof(double));
-  }
-  if (s->synthetic() && !s->general) {
-    A(s->m_W, nc * 6 * sizeof(double));
-    A(s->m_pr, nc * 6 * sizeof(double));
-    A(s->m_gW, nc * 18 * sizeof(double));
-    A(s->m_gP, nc * 15 * sizeof(double));
-    A(s->m_aux, nc * 4 * sizeof(double));
-    A(s->m_R, nc * 6 * sizeof(double));
-    A(s->m_invD, nc * 2 * sizeof(double));
-    A(s->d_ivol, nc * sizeof(double));
-    A(s->m_Fc, nc * 18 * sizeof(double));
-    A(s->m_corr, nc * 6 * sizeof(double));
-    A(s->m_gam, nc * 3 * sizeof(double));
-    A(s->m_Ffc, nc * 36 * sizeof(double));
-    A(s->m_G, nc * 72 * sizeof(double));
-    A(s->d_colnat, nc * sizeof(int));
-    A(s->m_wfl, (size_t)(s->nwall + 1) * 6 * sizeof(double));
-  }
+  // a synthetic solve's arrays, and those of the rectilinear one
+  auto solve = [&](auto &ptr, size_t bytes) {
+    if (s->synthetic()) A(ptr, bytes);
+  };
+  auto rect = [&](auto &ptr, size_t bytes) {
+    if (!s->general) solve(ptr, bytes);
+  };
+  rect(s->m_W, nc * 6 * sizeof(double));
+  rect(s->m_pr, nc * 6 * sizeof(double));
+  rect(s->m_gW, nc * 18 * sizeof(double));
+  rect(s->m_gP, nc * 15 * sizeof(double));
+  rect(s->m_aux, nc * 4 * sizeof(double));
+  solve(s->d_colcells, nc * sizeof(int));
+  rect(s->m_R, nc * 6 * sizeof(double));
+  rect(s->m_invD, nc * 2 * sizeof(double));
+  rect(s->d_ivol, nc * sizeof(double));
+  rect(s->m_Fc, nc * 18 * sizeof(double));
+  rect(s->m_corr, nc * 6 * sizeof(double));
+  rect(s->m_gam, nc * 3 * sizeof(double));
+  rect(s->m_Ffc, nc * 36 * sizeof(double));
+  solve(s->m_vis, nc * 3 * sizeof(double));
+  rect(s->m_G, nc * 72 * sizeof(double));
+  rect(s->d_colnat, nc * sizeof(int));
+  rect(s->m_wfl, (size_t)(s->nwall + 1) * 6 * sizeof(double));
+  solve(s->m_red, ((size_t)3 * MACRO_MAX_GRID * 16 + 32) * sizeof(double));
 }
 
 template <typename T, typename S>
